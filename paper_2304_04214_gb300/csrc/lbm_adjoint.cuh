@@ -592,7 +592,7 @@ __device__ __forceinline__ void collide_adjoint2(const V2 (&lam)[19], const Pair
     // ---- forward values ----
     const V2 rho = P.rho, irho = vrcp(rho);
     const V2 rux = HAS_FORCE ? vfma(0.5f, Fx, P.jx) : P.jx, ruy = P.jy;
-    const V2 ruz = HAS_FORCE ? vfma(0.5f, Fz, P.jz) : P.jz;
+    const V2 ruz = HAS_FORCE ? vfma(0.5f, Fz, -P.mjz) : -P.mjz;
     const V2 ux = rux * irho, uy = ruy * irho, uz = ruz * irho;
     const V2 uxx = rux * ux, uyy = ruy * uy, uzz = ruz * uz;
     const V2 usq = (uxx + uyy) + uzz;
@@ -876,7 +876,7 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
         if (v.tn >= 1e-12f) {
             const float itn = rcp_approx(v.tn);
             v.ex = u2x * itn; v.ez = u2z * itn;
-            const float jx = l ? P.jx.y : P.jx.x, jz = l ? P.jz.y : P.jz.x, rw = l ? P.rho.y : P.rho.x;
+            const float jx = l ? P.jx.y : P.jx.x, jz = l ? -P.mjz.y : -P.mjz.x, rw = l ? P.rho.y : P.rho.x;
             const float uhat = (jx * v.ex + jz * v.ez) * rcp_approx(rw);
             v.sg = uhat < 0.0f ? -1.0f : 1.0f;
             // the forward step stored this step's solution of eq:u_tau_implicit
@@ -888,8 +888,8 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
     if (a.wall_model) {
         if (!is_wall) {
             const V2 ir = vrcp(P.rho);
-            sh[slot][0] = P.jx.x; sh[slot][1] = P.jz.x; sh[slot][2] = ir.x;
-            sh[slot + 1][0] = P.jx.y; sh[slot + 1][1] = P.jz.y; sh[slot + 1][2] = ir.y;
+            sh[slot][0] = P.jx.x; sh[slot][1] = -P.mjz.x; sh[slot][2] = ir.x;
+            sh[slot + 1][0] = P.jx.y; sh[slot + 1][1] = -P.mjz.y; sh[slot + 1][2] = ir.y;
         }
         __syncthreads();
         if (is_wall) {
@@ -913,7 +913,7 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
         float gk = 0.f, gB = 0.f;
         if (is_wall) {
             const float lFx[2] = {A.lFx.x, A.lFx.y}, lFz[2] = {A.lFz.x, A.lFz.y};
-            const float rw[2] = {P.rho.x, P.rho.y}, jxw[2] = {P.jx.x, P.jx.y}, jzw[2] = {P.jz.x, P.jz.y};
+            const float rw[2] = {P.rho.x, P.rho.y}, jxw[2] = {P.jx.x, P.jx.y}, jzw[2] = {-P.mjz.x, -P.mjz.y};
             const WallLane vl[2] = {wall_lane(0), wall_lane(1)};
             float dljx[2] = {0.f, 0.f}, dljz[2] = {0.f, 0.f}, dlrho[2] = {0.f, 0.f};
             float lj2x[2] = {0.f, 0.f}, lj2z[2] = {0.f, 0.f}, li2[2] = {0.f, 0.f};
