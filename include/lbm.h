@@ -144,8 +144,8 @@ int lbm_bind_memory(lbm_handle *h, void *dev_ptr, size_t bytes);
  * regularized inlet (steps 6-8) and the collision (step 15); the wall-row
  * kernel (rows 0 and ny-1, on a side stream forked from and joined back into
  * the handle's stream) does the same for the first off-wall cells with the
- * wall model (steps 9-14).  (Odd nx, or LBM_KERNEL_CELL: one kernel for all
- * rows.)
+ * wall model (steps 9-14).  (Lattices of at most 100,000 cells: one kernel for
+ * all rows, the same arithmetic.)
  * With CUDA graphs on (the default, lbm_set_graphs), whole periods of the STG
  * ring (64 steps where the inlet plane allows) that fit in n are launched as
  * one graph each, built the first time a period's launch state occurs; the
@@ -202,7 +202,8 @@ int lbm_set_stream(lbm_handle *h, void *cuda_stream);
 /* ---- step kernel variants (all compute the same step of Algorithm 1) ---- */
 #define LBM_KERNEL_AUTO    0  /* QUAD for the 16-bit storages and PAIR for FP32 where the
                                  grid allows, else PAIR (nx even), else CELL */
-#define LBM_KERNEL_CELL    1  /* one cell per thread, direct loads */
+#define LBM_KERNEL_CELL    1  /* any nx, scalar loads: one cell per thread (FP32), or two
+                                 cells a block's width apart with packed FP32x2 (16-bit) */
 #define LBM_KERNEL_PAIR    2  /* two x-adjacent cells per thread, packed FP32x2; nx even */
 #define LBM_KERNEL_STAGED  3  /* PAIR arithmetic with the pulled populations copied into
                                  shared memory by the tensor memory accelerator (a
@@ -213,8 +214,8 @@ int lbm_set_stream(lbm_handle *h, void *cuda_stream);
 
 /* Choose the kernel of later steps (also the forward and recomputed steps of
  * lbm_adjoint_step).  PAIR, QUAD and STAGED run the same arithmetic and give
- * bit-identical states; CELL evaluates the same collision one cell at a time
- * (the same formulas, a different FP32 operation order).  Errors: LBM_EINVAL
+ * bit-identical states; CELL evaluates the same collision (FP32: the same
+ * formulas one cell at a time, a different operation order).  Errors: LBM_EINVAL
  * for an unknown kind or a grid the kind does not support. */
 int lbm_set_step_kernel(lbm_handle *h, int kind);
 

@@ -27,7 +27,7 @@ struct AdjIn {
     float lFx, lFy, lFz;    // of the force density
 };
 
-// Forward recompute and reverse of collide_mrt<false, HAS_FORCE> (FP32, f not
+// Forward recompute and reverse of the collision of one cell (FP32, f not
 // shifted).  lam: dJ/df* of the cell.  (lux, luy, luz): direct dJ/du of the
 // physical velocity (objective seeds).  Output: A (adjoint of the inputs; the
 // identity part lam itself is added by the caller).
@@ -389,7 +389,7 @@ __device__ __forceinline__ void adjoint_cell(const AdjArgs &a, int i, int j, int
     float vx = 0.f, vy = 0.f, vz = 0.f, rin = 1.f;
     if (is_inlet) adjoint_inlet_forward(a, f, j, k, vx, vy, vz, rin);
     Pairs P;
-    make_pairs<false>(f, P);
+    make_pairs(f, P);
     const float f9 = f[9];
     // ---- wall model forward ----
     const bool bot = G.bot, top = G.top, is_wall = WALLBLOCK && a.wall_model && (bot || top);
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(128, LBM_ADJ_MINB) adjoint_kernel(const __grid
 
 // ---------------------------------------------------------------------------
 // Interior rows, two x-adjacent cells (i0, i0 + 1) per thread with packed FP32x2
-// arithmetic -- the reverse of collide_pairs2<false, false> and of the pull,
+// arithmetic -- the reverse of collide2 and of the pull,
 // the same chain as adjoint_cell written for two cells at once.  Only regular
 // pairs take this path: a pair holding the inlet cell, or a cell whose
 // populations the outlet's clamped pull reads twice, goes through
@@ -581,7 +581,7 @@ struct AdjIn2 {
     V2 lFx, lFz;            // of the wall force (F_y = 0: the force is wall-parallel)
 };
 
-// Reverse of collide_pairs2<false, HAS_FORCE> for two cells: lam = dJ/df*;
+// Reverse of collide2 (FP32 form, HAS_FORCE = forced) for two cells: lam = dJ/df*;
 // (lux, luy) direct dJ/du seeds; (Fx, 0, Fz) the wall force when HAS_FORCE.
 // A receives the adjoint of the collision's inputs (the identity part lam is
 // added by adjoint_to_pops2).
@@ -592,7 +592,7 @@ __device__ __forceinline__ void collide_adjoint2(const V2 (&lam)[19], const Pair
     // ---- forward values ----
     const V2 rho = P.rho, irho = vrcp(rho);
     const V2 rux = HAS_FORCE ? vfma(0.5f, Fx, P.jx) : P.jx, ruy = P.jy;
-    const V2 ruz = HAS_FORCE ? vfma(0.5f, Fz, -P.mjz) : -P.mjz;
+    const V2 ruz = HAS_FORCE ? vfma(0.5f, Fz, P.jz) : P.jz;
     const V2 ux = rux * irho, uy = ruy * irho, uz = ruz * irho;
     const V2 uxx = rux * ux, uyy = ruy * uy, uzz = ruz * uz;
     const V2 usq = (uxx + uyy) + uzz;
@@ -613,7 +613,7 @@ __device__ __forceinline__ void collide_adjoint2(const V2 (&lam)[19], const Pair
     const V2 Qh = vsqrt(qq);
     const V2 Rr = vsqrt(vfma(csm18 * Qh, irho, tau0 * tau0));
     const V2 sv = 2.0f * vrcp(tau0 + Rr);
-    // Guo source moments with F_y = 0 (collide_pairs2)
+    // Guo source moments with F_y = 0 (collide2)
     V2 F9 = vdup(0.0f), F11 = vdup(0.0f), F13 = vdup(0.0f), F14 = vdup(0.0f), F15 = vdup(0.0f);
     if (HAS_FORCE) {
         F9 = vfma(4.0f, ux * Fx, -2.0f * (uz * Fz));
@@ -829,7 +829,7 @@ __device__ __forceinline__ void adjoint_pair(const AdjArgs &a, int i0, int j, in
 #pragma unroll
     for (int q = 0; q < 19; ++q) lam[q] = *reinterpret_cast<const float2 *>(a.lam + q * N + c);
     Pairs2 P;
-    make_pairs2<false>(f, P);
+    make_pairs2(f, P);
     V2 lux, luy;
     jr_seeds2(a, P, vdup(0.0f), i0, j, lux, luy);
     AdjIn2 A;
@@ -862,7 +862,7 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
 #pragma unroll
     for (int q = 0; q < 19; ++q) lam[q] = *reinterpret_cast<const float2 *>(a.lam + q * N + c);
     Pairs2 P;
-    make_pairs2<false>(f, P);
+    make_pairs2(f, P);
     // ---- wall model forward (eq:base, eq:uhat, this step's u_tau, eq:force_wm) ----
     // Per lane from u_2 (in sh), the cell's momentum and density and this
     // step's u_tau; evaluated for the force here and again in the reverse
@@ -876,7 +876,7 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
         if (v.tn >= 1e-12f) {
             const float itn = rcp_approx(v.tn);
             v.ex = u2x * itn; v.ez = u2z * itn;
-            const float jx = l ? P.jx.y : P.jx.x, jz = l ? -P.mjz.y : -P.mjz.x, rw = l ? P.rho.y : P.rho.x;
+            const float jx = l ? P.jx.y : P.jx.x, jz = l ? P.jz.y : P.jz.x, rw = l ? P.rho.y : P.rho.x;
             const float uhat = (jx * v.ex + jz * v.ez) * rcp_approx(rw);
             v.sg = uhat < 0.0f ? -1.0f : 1.0f;
             // the forward step stored this step's solution of eq:u_tau_implicit
@@ -888,8 +888,8 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
     if (a.wall_model) {
         if (!is_wall) {
             const V2 ir = vrcp(P.rho);
-            sh[slot][0] = P.jx.x; sh[slot][1] = -P.mjz.x; sh[slot][2] = ir.x;
-            sh[slot + 1][0] = P.jx.y; sh[slot + 1][1] = -P.mjz.y; sh[slot + 1][2] = ir.y;
+            sh[slot][0] = P.jx.x; sh[slot][1] = P.jz.x; sh[slot][2] = ir.x;
+            sh[slot + 1][0] = P.jx.y; sh[slot + 1][1] = P.jz.y; sh[slot + 1][2] = ir.y;
         }
         __syncthreads();
         if (is_wall) {
@@ -913,7 +913,7 @@ __device__ __forceinline__ void adjoint_wall_pair(const AdjArgs &a, int i0, int 
         float gk = 0.f, gB = 0.f;
         if (is_wall) {
             const float lFx[2] = {A.lFx.x, A.lFx.y}, lFz[2] = {A.lFz.x, A.lFz.y};
-            const float rw[2] = {P.rho.x, P.rho.y}, jxw[2] = {P.jx.x, P.jx.y}, jzw[2] = {-P.mjz.x, -P.mjz.y};
+            const float rw[2] = {P.rho.x, P.rho.y}, jxw[2] = {P.jx.x, P.jx.y}, jzw[2] = {P.jz.x, P.jz.y};
             const WallLane vl[2] = {wall_lane(0), wall_lane(1)};
             float dljx[2] = {0.f, 0.f}, dljz[2] = {0.f, 0.f}, dlrho[2] = {0.f, 0.f};
             float lj2x[2] = {0.f, 0.f}, lj2z[2] = {0.f, 0.f}, li2[2] = {0.f, 0.f};

@@ -15,6 +15,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "lbm.h"
@@ -712,6 +713,16 @@ void sponge_args(const lbm_handle *h, float &x0, float &inv, float &s3nu) {
     s3nu = L > 0 ? (float)(3.0 * h->sponge_nu) : 0.0f;
 }
 
+// Whether a step runs as one launch, wall blocks and interior blocks together,
+// or as an interior kernel with the wall rows on a side stream beside it.  Up to
+// about 100,000 cells all blocks of the one launch are resident at once and it
+// saves the fork and join (64x32x32: FP32 5.1 -> 4.4 us per step in a graph, FP16
+// 5.4 -> 4.8); beyond that the wall blocks, whose chain is the longer one, hold
+// up the interior ones that wait for their place (96x32x48: FP32 6.0 -> 6.5 us;
+// 400x40x32: 11.6 -> 12.6).
+constexpr long long kOneLaunchCells = 100000;
+bool one_launch(const lbm_handle *h) { return h->ncell <= kOneLaunchCells; }
+
 template <class S>
 cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
     using T = typename S::T;
@@ -740,7 +751,6 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
     a.kappa = (float)h->theta[2]; a.B = (float)h->theta[3];
     a.obj = io.obj; a.obj_i0 = io.obj_i0; a.obj_i1 = io.obj_i1; a.obj_iR = io.obj_iR;
     sponge_args(h, a.sp_x0, a.sp_inv, a.sp_3nu);
-    const int bxmax = lbmk::STEP_THREADS / lbmk::BY;
     // (steps inside a graph are timed by events around the graph launch)
     const bool timed = h->prof_on && !h->capturing && (h->prof_count++ % h->prof_every) == 0;
     cudaEvent_t tev0 = nullptr, tev1 = nullptr;
@@ -752,14 +762,37 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
     if (timed) cudaEventRecord(tev0, h->stream);
     int kind = resolve_kind(h);
     if (io.obj && kind != LBM_KERNEL_CELL) kind = LBM_KERNEL_PAIR;   // the kernel that sums the objective
-    if (io.fw == h->d_fw) h->fw_side = kind != LBM_KERNEL_CELL;
+    // block (bx, BY), two cells a thread: 2 bx columns of two rows; bx = 32 where
+    // it covers the row with fewer empty columns (400 columns: 448 instead of 512,
+    // 11.4 -> 10.8 us per 400x40x32 FP32 step)
+    const int n32 = (h->nx + 63) / 64, wide = lbmk::STEP_THREADS / lbmk::BY;
+    const int bx = n32 % (wide / 32) ? 32 : wide;
+    const int nbx = (h->nx + 2 * bx - 1) / (2 * bx);
+    const dim3 block(bx, lbmk::BY);
+    const bool split = h->nx % 2 != 0 || kind == LBM_KERNEL_CELL;
+    const bool one = kind != LBM_KERNEL_STAGED && one_launch(h);
+    constexpr bool fp32 = std::is_same<S, lbmk::StoreF32>::value;
     cudaError_t err = cudaSuccess;
-    if (kind == LBM_KERNEL_STAGED || kind == LBM_KERNEL_PAIR || kind == LBM_KERNEL_QUAD) {
+    const bool cell32 = fp32 && kind == LBM_KERNEL_CELL;
+    if (io.fw == h->d_fw) h->fw_side = !one;
+    if (cell32 && one) {
+        if constexpr (fp32) {
+            const dim3 grid((h->nx + 31) / 32, h->ny / lbmk::BY, h->nz), cblock(32, lbmk::BY);
+            if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_ALL><<<grid, cblock, 0, h->stream>>>(a);
+            else lbmk::step_kernel<false, lbmk::CELLS_ALL><<<grid, cblock, 0, h->stream>>>(a);
+        }
+    } else if (one) {
+        const dim3 grid(nbx, h->ny / lbmk::BY, h->nz);
+        if (!split) {
+            if (io.stats) lbmk::step2_kernel<S, true, false, true><<<grid, block, 0, h->stream>>>(a);
+            else lbmk::step2_kernel<S, false, false, true><<<grid, block, 0, h->stream>>>(a);
+        } else if constexpr (!fp32) {
+            if (io.stats) lbmk::step2_kernel<S, true, true, true><<<grid, block, 0, h->stream>>>(a);
+            else lbmk::step2_kernel<S, false, true, true><<<grid, block, 0, h->stream>>>(a);
+        }
+    } else {
         // the wall rows on the side stream, the interior rows on the handle's
         // stream; both read the state of the previous step and write disjoint rows
-        const int bx = (h->nx / 2) >= bxmax ? bxmax : 32;
-        const int nbx = (h->nx / 2 + bx - 1) / bx;
-        const dim3 block(bx, lbmk::BY);
         if ((err = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess ||
             (err = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess)
             return err;
@@ -770,28 +803,41 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
         a.wall_planes = std::max(1, std::min(4, (int)(interior_us / 12.0)));
         const dim3 wgrid((h->nx + lbmk::WALL_THREADS - 1) / lbmk::WALL_THREADS,
                          (h->nz + a.wall_planes - 1) / a.wall_planes);
-        if (io.stats) lbmk::wall_kernel<S, true><<<wgrid, lbmk::WALL_THREADS, 0, h->side>>>(a);
+        const int cx = h->nx >= 64 ? 64 : 32;
+        const dim3 cgrid((h->nx + cx - 1) / cx, h->ny / lbmk::BY, h->nz), cblock(cx, lbmk::BY);
+        if (cell32) {
+            if constexpr (fp32) {
+                const dim3 cw(cgrid.x, 2, cgrid.z);
+                if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_WALL><<<cw, cblock, 0, h->side>>>(a);
+                else lbmk::step_kernel<false, lbmk::CELLS_WALL><<<cw, cblock, 0, h->side>>>(a);
+            }
+        } else if (io.stats) lbmk::wall_kernel<S, true><<<wgrid, lbmk::WALL_THREADS, 0, h->side>>>(a);
         else lbmk::wall_kernel<S, false><<<wgrid, lbmk::WALL_THREADS, 0, h->side>>>(a);
         if ((err = cudaEventRecord(h->ev_join, h->side)) != cudaSuccess) return err;
-        if (kind == LBM_KERNEL_STAGED) {
+        const dim3 grid(nbx, (h->ny - 2) / lbmk::BY, h->nz);
+        if (cell32) {
+            if constexpr (fp32) {
+                const dim3 ci(cgrid.x, cgrid.y - 2, cgrid.z);
+                if (ci.y == 0) { /* ny = 4: wall rows only */ }
+                else if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_INTERIOR><<<ci, cblock, 0, h->stream>>>(a);
+                else lbmk::step_kernel<false, lbmk::CELLS_INTERIOR><<<ci, cblock, 0, h->stream>>>(a);
+            }
+        } else if (kind == LBM_KERNEL_STAGED) {
             err = io.stats ? launch_staged<S, true>(h, a, io.in) : launch_staged<S, false>(h, a, io.in);
         } else if (kind == LBM_KERNEL_QUAD) {
             const dim3 qgrid((h->nx + 127) / 128, (h->ny - 2) / lbmk::BY, h->nz), qblock(32, lbmk::BY);
             if (io.stats) lbmk::step4_kernel<S, true><<<qgrid, qblock, 0, h->stream>>>(a);
             else lbmk::step4_kernel<S, false><<<qgrid, qblock, 0, h->stream>>>(a);
-        } else {
-            const dim3 grid(nbx, (h->ny - 2) / lbmk::BY, h->nz);
-            if (io.stats) lbmk::step2_kernel<S, true><<<grid, block, 0, h->stream>>>(a);
-            else lbmk::step2_kernel<S, false><<<grid, block, 0, h->stream>>>(a);
+        } else if (!split) {
+            if (io.stats) lbmk::step2_kernel<S, true, false, false><<<grid, block, 0, h->stream>>>(a);
+            else lbmk::step2_kernel<S, false, false, false><<<grid, block, 0, h->stream>>>(a);
+        } else if constexpr (!fp32) {
+            if (io.stats) lbmk::step2_kernel<S, true, true, false><<<grid, block, 0, h->stream>>>(a);
+            else lbmk::step2_kernel<S, false, true, false><<<grid, block, 0, h->stream>>>(a);
         }
         cudaError_t e2 = cudaStreamWaitEvent(h->stream, h->ev_join, 0);
         if (err == cudaSuccess) err = e2;
         h->launches += 1;
-    } else {
-        const int bx = h->nx >= bxmax ? bxmax : (h->nx >= 64 && bxmax >= 64 ? 64 : 32);
-        dim3 block(bx, lbmk::BY), grid((h->nx + bx - 1) / bx, h->ny / lbmk::BY, h->nz);
-        if (io.stats) lbmk::step_kernel<S, true><<<grid, block, 0, h->stream>>>(a);
-        else lbmk::step_kernel<S, false><<<grid, block, 0, h->stream>>>(a);
     }
     if (timed) cudaEventRecord(tev1, h->stream);
     h->launches += 1;
