@@ -267,7 +267,6 @@ struct lbm_handle {
             }
         }
     }
-    float rb(int j, int q) const { return rowbase[(size_t)j * lbmk::RB_W + q]; }
 
     // Flow constants (A20): U_b+ = mean of u+ over the cell centres with the
     // creation-time (kappa, B); u_tau = U_b / U_b+, nu = u_tau delta / Re_tau.
@@ -1022,23 +1021,6 @@ void launch_init(lbm_handle *h, void *lat) {
                                                                                h->d_rowbase, h->nx, h->ny, n);
 }
 
-const double kW[19] = {1. / 36, 1. / 36, 1. / 18, 1. / 36, 1. / 36, 1. / 36, 1. / 18, 1. / 36, 1. / 18, 1. / 3,
-                       1. / 18, 1. / 36, 1. / 18, 1. / 36, 1. / 36, 1. / 36, 1. / 18, 1. / 36, 1. / 36};
-
-uint16_t f32_to_bf16_rn(float x) {
-    uint32_t b;
-    std::memcpy(&b, &x, 4);
-    if ((b & 0x7f800000u) == 0x7f800000u) return (uint16_t)(b >> 16);   // inf / nan
-    b += 0x7fffu + ((b >> 16) & 1u);
-    return (uint16_t)(b >> 16);
-}
-float bf16_to_f32(uint16_t v) {
-    uint32_t b = (uint32_t)v << 16;
-    float x;
-    std::memcpy(&x, &b, 4);
-    return x;
-}
-
 // ---------------------------------------------------------------------------
 // CUDA graphs of whole STG ring periods.  lbm_step launches the stg_ring steps
 // that start where the ring swaps halves as one graph: the steps of one
@@ -1191,6 +1173,41 @@ int graph_segment(lbm_handle *h) {
     h->fw_side = false;
     ++h->graph_launches;
     return LBM_OK;
+}
+
+// Host FP64 arrays of populations ([19][ncell]) to and from a lattice of stored
+// words: converted on the device through the lattice buffer that is free
+// between steps, a chunk of as many values as it holds at a time.
+template <class S>
+cudaError_t pops_copy_t(lbm_handle *h, typename S::T *f, double *out, const double *in) {
+    const long long n = 19 * h->ncell, chunk = (long long)(19 * (size_t)h->ncell * h->elem / sizeof(double));
+    double *scratch = (double *)h->lat[h->cur ^ 1];
+    for (long long i = 0; i < n; i += chunk) {
+        const long long c = std::min(chunk, n - i);
+        const unsigned blocks = (unsigned)((c + 255) / 256);
+        cudaError_t e;
+        if (in && (e = cudaMemcpyAsync(scratch, in + i, c * sizeof(double), cudaMemcpyHostToDevice, h->stream)) !=
+                      cudaSuccess)
+            return e;
+        if (in) lbmk::pops_from_f64_kernel<S><<<blocks, 256, 0, h->stream>>>(f, h->d_rowbase, scratch, i, c, h->nx,
+                                                                             h->ny, h->ncell);
+        else lbmk::pops_to_f64_kernel<S><<<blocks, 256, 0, h->stream>>>(f, h->d_rowbase, scratch, i, c, h->nx, h->ny,
+                                                                        h->ncell);
+        h->launches += 1;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (out && (e = cudaMemcpyAsync(out + i, scratch, c * sizeof(double), cudaMemcpyDeviceToHost, h->stream)) !=
+                       cudaSuccess)
+            return e;
+    }
+    return cudaStreamSynchronize(h->stream);
+}
+cudaError_t pops_copy(lbm_handle *h, void *f, double *out, const double *in) {
+    switch (h->opts.precision) {
+        case LBM_FP16_DEV: return pops_copy_t<lbmk::StoreF16>(h, (__half *)f, out, in);
+        case LBM_BF16_DEV: return pops_copy_t<lbmk::StoreBF16>(h, (__nv_bfloat16 *)f, out, in);
+        case LBM_FP16_ROW: return pops_copy_t<lbmk::StoreF16R>(h, (__half *)f, out, in);
+        default: return pops_copy_t<lbmk::StoreF32>(h, (float *)f, out, in);
+    }
 }
 
 }  // namespace
@@ -1522,9 +1539,9 @@ int lbm_get_fields(lbm_handle *h, double *rho, double *u) {
     if (!h || !rho || !u) return LBM_EINVAL;
     LBM_DEVICE_GUARD(h);
     if (!h->bound) return LBM_ESTATE;
-    // the other lattice is free between steps: use it as scratch (>= 16 B per cell)
-    float *drho = (float *)h->lat[h->cur ^ 1];
-    float *du = drho + h->ncell;
+    // the other lattice is free between steps: use it as scratch (>= 32 B per cell)
+    double *drho = (double *)h->lat[h->cur ^ 1];
+    double *du = drho + h->ncell;
     const long long n = h->ncell;
     const unsigned blocks = (unsigned)((n + 255) / 256);
     h->launches += 1;
@@ -1547,62 +1564,24 @@ int lbm_get_fields(lbm_handle *h, double *rho, double *u) {
     }
     cudaError_t e;
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e);
-    std::vector<float> buf(4 * (size_t)n);
-    if ((e = cudaMemcpyAsync(buf.data(), drho, 4 * sizeof(float) * n, cudaMemcpyDeviceToHost, h->stream)) !=
-        cudaSuccess) return cuda_fail(e);
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(e);
-    for (long long c = 0; c < n; ++c) rho[c] = buf[c];
-    for (long long c = 0; c < 3 * n; ++c) u[c] = buf[n + c];
-    return LBM_OK;
+    if ((e = cudaMemcpyAsync(rho, drho, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(u, du, 3 * sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
+        return cuda_fail(e);
+    return cuda_fail(cudaStreamSynchronize(h->stream));
 }
 
 int lbm_get_populations(lbm_handle *h, double *f) {
     if (!h || !f) return LBM_EINVAL;
     LBM_DEVICE_GUARD(h);
     if (!h->bound) return LBM_ESTATE;
-    const size_t n = 19 * (size_t)h->ncell;
-    std::vector<char> buf(n * h->elem);
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(buf.data(), h->lat[h->cur], n * h->elem, cudaMemcpyDeviceToHost, h->stream)) !=
-        cudaSuccess) return cuda_fail(e);
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(e);
-    const size_t N = h->ncell;
-    for (size_t idx = 0; idx < n; ++idx) {
-        const int q = (int)(idx / N);
-        if (h->opts.precision == LBM_FP32) f[idx] = ((const float *)buf.data())[idx];
-        else if (h->opts.precision == LBM_FP16_DEV)
-            f[idx] = kW[q] + (double)__half2float(((const __half *)buf.data())[idx]);
-        else {  // row base: f - w as the kernels form it, stored word + row base, in FP32
-            const float word = h->opts.precision == LBM_BF16_DEV
-                                   ? bf16_to_f32(((const uint16_t *)buf.data())[idx])
-                                   : __half2float(((const __half *)buf.data())[idx]);
-            f[idx] = kW[q] + (double)(word + h->rb((int)((idx % N) / h->nx % h->ny), q));
-        }
-    }
-    return LBM_OK;
+    return cuda_fail(pops_copy(h, h->lat[h->cur], f, nullptr));
 }
 
 int lbm_set_populations(lbm_handle *h, const double *f) {
     if (!h || !f) return LBM_EINVAL;
     LBM_DEVICE_GUARD(h);
     if (!h->bound) return LBM_ESTATE;
-    const size_t n = 19 * (size_t)h->ncell, N = h->ncell;
-    std::vector<char> buf(n * h->elem);
-    for (size_t idx = 0; idx < n; ++idx) {
-        const int q = (int)(idx / N);
-        if (h->opts.precision == LBM_FP32) ((float *)buf.data())[idx] = (float)f[idx];
-        else if (h->opts.precision == LBM_FP16_DEV)
-            ((__half *)buf.data())[idx] = __double2half(f[idx] - kW[q]);
-        else {
-            const float dev = (float)(f[idx] - kW[q] - (double)h->rb((int)((idx % N) / h->nx % h->ny), q));
-            if (h->opts.precision == LBM_BF16_DEV) ((uint16_t *)buf.data())[idx] = f32_to_bf16_rn(dev);
-            else ((__half *)buf.data())[idx] = __float2half_rn(dev);
-        }
-    }
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(h->lat[h->cur], buf.data(), n * h->elem, cudaMemcpyHostToDevice, h->stream)) !=
-        cudaSuccess) return cuda_fail(e);
-    return cuda_fail(cudaStreamSynchronize(h->stream));
+    return cuda_fail(pops_copy(h, h->lat[h->cur], nullptr, f));
 }
 
 int lbm_get_utau(lbm_handle *h, double *utau) {
@@ -2113,14 +2092,7 @@ int lbm_adjoint_state_gradient(lbm_handle *h, double *lambda0) {
     if (!h || !lambda0) return LBM_EINVAL;
     LBM_DEVICE_GUARD(h);
     if (!h->adj.bound || !h->adj.have_lambda0) return LBM_ESTATE;
-    const size_t L = 19 * (size_t)h->ncell;
-    std::vector<float> buf(L);
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(buf.data(), h->adj.lamA, L * 4, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
-        return cuda_fail(e);
-    if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) return cuda_fail(e);
-    for (size_t c = 0; c < L; ++c) lambda0[c] = buf[c];
-    return LBM_OK;
+    return cuda_fail(pops_copy(h, h->adj.lamA, lambda0, nullptr));
 }
 
 int lbm_vjp_step(lbm_handle *h, const double *lambda_next, double *lambda_prev, double dtheta[4]) {
@@ -2144,21 +2116,15 @@ int lbm_vjp_step(lbm_handle *h, const double *lambda_next, double *lambda_prev, 
     io.in = h->lat[h->cur]; io.out = A.lamB; io.utau = A.ut_scr; io.fw = A.fw_scr; io.vprime = A.vwin;
     io.stats = false;
     if (cudaError_t le = launch_step_io(h, io)) return cuda_fail(le);
-    std::vector<float> buf(L);
-    for (size_t c = 0; c < L; ++c) buf[c] = (float)lambda_next[c];
-    if ((e = cudaMemcpyAsync(A.lamA, buf.data(), L * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess)
-        return cuda_fail(e);
+    if ((e = pops_copy(h, A.lamA, nullptr, lambda_next)) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemsetAsync(A.lamB, 0, L * 4, st)) != cudaSuccess) return cuda_fail(e);
     launch_adjoint(h, (const float *)h->lat[h->cur], A.lamA, A.lamB, A.ut_scr, A.vwin,
                    h->opts.inlet ? A.luin : nullptr, false, nullptr, 0.0f);
     launch_stg_adjoint(h, h->t, 1, h->adj.luin, h->stream);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(buf.data(), A.lamB, L * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-        return cuda_fail(e);
     if ((e = cudaMemcpyAsync(dtheta, A.gtheta, 4 * sizeof(double), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
         return cuda_fail(e);
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e);
-    for (size_t c = 0; c < L; ++c) lambda_prev[c] = buf[c];
+    if ((e = pops_copy(h, A.lamB, lambda_prev, nullptr)) != cudaSuccess) return cuda_fail(e);
     A.have_lambda0 = false;
     return LBM_OK;
 }
