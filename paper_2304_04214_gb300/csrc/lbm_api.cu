@@ -83,7 +83,7 @@ inline Dual operator/(Dual a, Dual b) { return {a.v / b.v, (a.d * b.v - a.v * b.
 inline Dual dexp(Dual a) { const double e = std::exp(a.v); return {e, e * a.d}; }
 inline Dual dsqrt(Dual a) { const double r = std::sqrt(a.v); return {r, a.d / (2.0 * r)}; }
 inline Dual dtanh(Dual a) { const double t = std::tanh(a.v); return {t, (1.0 - t * t) * a.d}; }
-inline Dual dpow(Dual a, double e) { const double p = std::pow(a.v, e); return {p, e * std::pow(a.v, e - 1.0) * a.d}; }
+inline Dual dpow(Dual a, double e) { const double p = std::pow(a.v, e); return {p, e * p / a.v * a.d}; }
 inline double dexp(double a) { return std::exp(a); }
 inline double dsqrt(double a) { return std::sqrt(a); }
 inline double dtanh(double a) { return std::tanh(a); }
@@ -378,7 +378,8 @@ struct lbm_handle {
         const T kmin = T(beta_kmin * 2.0 * kPi) / mx;
         const double kcut = kPi;
         out.assign((size_t)ny * N, T(0.0));
-        std::vector<T> E(N);
+        std::vector<T> E(N), kn(N);
+        for (int n = 0; n < N; ++n) kn[n] = kmin * T(std::pow(k_ratio, n));   // not per row
         for (int j = 0; j < ny; ++j) {
             const double d = dwall(j);
             const T ke = T(2.0 * kPi) / ell[j];
@@ -386,15 +387,16 @@ struct lbm_handle {
             const double keta = 2.0 * kPi * std::pow(eps / (nu * nu * nu), 0.25);
             T tot(0.0);
             for (int n = 0; n < N; ++n) {
-                const T k = kmin * T(std::pow(k_ratio, n));
+                const T k = kn[n];
                 const T r = k / ke;
                 const T dk = k * T(1.0 - 1.0 / k_ratio);
-                const double over = std::max(val(k) - 0.9 * kcut, 0.0);
-                T xc = val(k) > 0.9 * kcut ? T(4.0) * (k - T(0.9 * kcut)) / T(kcut) : T(0.0);
-                (void)over;
                 const T g = T(12.0) * k / T(keta);
-                E[n] = r * r * r * r / dpow(T(1.0) + T(2.4) * r * r, 17.0 / 6.0) * dexp(T(0.0) - g * g) *
-                       dexp(T(0.0) - xc * xc * xc) * dk;
+                E[n] = r * r * r * r / dpow(T(1.0) + T(2.4) * r * r, 17.0 / 6.0) * dexp(T(0.0) - g * g);
+                if (val(k) > 0.9 * kcut) {          // the grid cut-off (1 below it)
+                    const T xc = T(4.0) * (k - T(0.9 * kcut)) / T(kcut);
+                    E[n] = E[n] * dexp(T(0.0) - xc * xc * xc);
+                }
+                E[n] = E[n] * dk;
                 tot = tot + E[n];
             }
             for (int n = 0; n < N; ++n) out[(size_t)j * N + n] = dsqrt(T(6.0) * E[n] / tot);
