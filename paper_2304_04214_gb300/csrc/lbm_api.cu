@@ -827,8 +827,15 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
             err = io.stats ? launch_staged<S, true>(h, a, io.in) : launch_staged<S, false>(h, a, io.in);
         } else if (kind == LBM_KERNEL_QUAD) {
             const dim3 qgrid((h->nx + 127) / 128, (h->ny - 2) / lbmk::BY, h->nz), qblock(32, lbmk::BY);
-            if (io.stats) lbmk::step4_kernel<S, true><<<qgrid, qblock, 0, h->stream>>>(a);
-            else lbmk::step4_kernel<S, false><<<qgrid, qblock, 0, h->stream>>>(a);
+            if (io.stats) lbmk::step4_kernel<S, true, false><<<qgrid, qblock, 0, h->stream>>>(a);
+            else lbmk::step4_kernel<S, false, false><<<qgrid, qblock, 0, h->stream>>>(a);
+        } else if (!fp32 && !split && h->nx % 4 != 0) {
+            // 16-bit words are worth four cells a thread also where rows start on a pair
+            if constexpr (!fp32) {
+                const dim3 qgrid((h->nx + 127) / 128, (h->ny - 2) / lbmk::BY, h->nz), qblock(32, lbmk::BY);
+                if (io.stats) lbmk::step4_kernel<S, true, true><<<qgrid, qblock, 0, h->stream>>>(a);
+                else lbmk::step4_kernel<S, false, true><<<qgrid, qblock, 0, h->stream>>>(a);
+            }
         } else if (!split) {
             if (io.stats) lbmk::step2_kernel<S, true, false, false><<<grid, block, 0, h->stream>>>(a);
             else lbmk::step2_kernel<S, false, false, false><<<grid, block, 0, h->stream>>>(a);

@@ -91,3 +91,26 @@ def test_newton_from_far_above_the_root(kernel, nx):
     else:
         r = g.utau() / uo
         assert 0.5 < r.min() and r.max() < 2.0
+
+
+@pytest.mark.parametrize("inlet", [1, 0])
+@pytest.mark.parametrize("precision,tol", [("fp16", 1.5e-3), ("bf16", 1.2e-2), ("fp16row", 1.5e-3)])
+@pytest.mark.parametrize("shape", [(1026, 8, 14), (898, 10, 12), (126, 30, 28), (130, 30, 28)])
+def test_rows_of_pairs_match_the_oracle(shape, precision, tol, inlet):
+    """16-bit lattices above 100,000 cells with nx = 4m + 2: the last thread of a row has
+    one pair of cells, alone in its warp (1026, 130), at a warp's end (126) or within
+    one (898).  Two steps with statistics: fields to the two-step tolerance,
+    statistics sums per summed term as in the parity tests."""
+    nx, ny, nz = shape
+    assert nx % 4 == 2 and nx * ny * nz > 100000
+    o, g = make_pair(nx, ny, nz, n_modes=8, seed=6, precision=precision, inlet=inlet, stats=1)
+    assert g.step_kernel == "pair"
+    set_both(o, g, o.state() * (1.0 + 0.02 * noise((19, nz, ny, nx), seed=8)))
+    o.step(2)
+    g.step(2)
+    g.sync()
+    er, eu = field_errors(o, g)
+    assert er < tol and eu < tol, (er, eu)
+    su = g.stats()[0][..., 0]
+    _, uo = o.fields()
+    assert np.max(np.abs(su - o.stats()[0].reshape(ny, nx, 7)[..., 0])) < 2 * nz * tol * np.max(np.abs(uo))
