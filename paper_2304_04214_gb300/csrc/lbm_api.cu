@@ -195,6 +195,7 @@ struct lbm_handle {
     // ev_prof_ready[b]: the upload into buffer b is done (and its staging half
     // free); ev_prof_free[b]: the steps that read buffer b are done
     float *pin_stage = nullptr;
+    double *pin_shear = nullptr;           // behind it, [2][nx]: lbm_wall_shear's kernel writes here
     cudaStream_t copy = nullptr;
     cudaEvent_t ev_prof_ready[2] = {nullptr, nullptr}, ev_prof_free[2] = {nullptr, nullptr};
     // instrumentation
@@ -1310,7 +1311,9 @@ int lbm_bind_memory(lbm_handle *h, void *dev_ptr, size_t bytes) {
     h->mem_bytes = need;
     int prio_lo = 0, prio_hi = 0;
     cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
-    if (cudaHostAlloc((void **)&h->pin_stage, 14 * sizeof(float) * h->ny, cudaHostAllocDefault) != cudaSuccess ||
+    const size_t stage_bytes = 14 * sizeof(float) * h->ny;               // (a multiple of 8: ny is even)
+    if (cudaHostAlloc((void **)&h->pin_stage, stage_bytes + 2 * sizeof(double) * h->nx, cudaHostAllocDefault) !=
+            cudaSuccess ||
         cudaStreamCreateWithFlags(&h->copy, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_prof_ready[0], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_prof_ready[1], cudaEventDisableTiming) != cudaSuccess ||
@@ -1329,6 +1332,7 @@ int lbm_bind_memory(lbm_handle *h, void *dev_ptr, size_t bytes) {
         h->mem = nullptr;
         return cuda_fail(cudaGetLastError());
     }
+    h->pin_shear = (double *)((char *)h->pin_stage + stage_bytes);
     Arena ar;
     ar.base = (char *)h->mem;
     ar.guard = h->guard_bytes;
@@ -1747,9 +1751,14 @@ int lbm_wall_shear_async(lbm_handle *h, double *out) {
 int lbm_wall_shear(lbm_handle *h, double *out) {
     if (!h || !out) return LBM_EINVAL;
     LBM_DEVICE_GUARD(h);
-    const int rc = lbm_wall_shear_async(h, out);
+    if (!h->bound) return LBM_ESTATE;
+    // through the handle's page-locked buffer, which the reduction writes itself:
+    // no copy on the stream into the caller's pageable array
+    const int rc = lbm_wall_shear_async(h, h->pin_shear);
     if (rc) return rc;
-    return cuda_fail(cudaStreamSynchronize(h->stream));
+    const cudaError_t e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) std::copy(h->pin_shear, h->pin_shear + 2 * (size_t)h->nx, out);
+    return cuda_fail(e);
 }
 
 // ---------------------------------------------------------------------------
