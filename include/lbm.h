@@ -215,8 +215,11 @@ int lbm_set_stream(lbm_handle *h, void *cuda_stream);
 /* Choose the kernel of later steps (also the forward and recomputed steps of
  * lbm_adjoint_step).  PAIR, QUAD and STAGED run the same arithmetic and give
  * bit-identical states; CELL evaluates the same collision (FP32: the same
- * formulas one cell at a time, a different operation order).  Errors: LBM_EINVAL
- * for an unknown kind or a grid the kind does not support. */
+ * formulas one cell at a time, a different operation order).  Lattices of at
+ * most 100,000 cells run PAIR, QUAD and the 16-bit CELL as the two-cell kernel in
+ * one launch, and 16-bit PAIR steps of larger ones with nx = 4m + 2 take four
+ * cells per thread: the same bits.  Errors: LBM_EINVAL for an unknown kind or a
+ * grid the kind does not support. */
 int lbm_set_step_kernel(lbm_handle *h, int kind);
 
 /* The kernel later steps will run (AUTO resolved) into *kind.  Errors:
