@@ -213,16 +213,20 @@ int lbm_set_stream(lbm_handle *h, void *cuda_stream);
                                  shuffle, PAIR arithmetic; nx a multiple of 4 */
 
 /* Choose the kernel of later steps (also the forward and recomputed steps of
- * lbm_adjoint_step).  PAIR, QUAD and STAGED run the same arithmetic and give
- * bit-identical states; CELL evaluates the same collision (FP32: the same
- * formulas one cell at a time, a different operation order).  Lattices of at
- * most 100,000 cells run PAIR, QUAD and the 16-bit CELL as the two-cell kernel in
- * one launch, and 16-bit PAIR steps of larger ones with nx = 4m + 2 take four
- * cells per thread: the same bits.  Errors: LBM_EINVAL for an unknown kind or a
- * grid the kind does not support. */
+ * lbm_adjoint_step, except that PAIR's kernel sums the objective of a window's
+ * forward steps where QUAD or STAGED is chosen).  PAIR, QUAD and STAGED run the
+ * same arithmetic and give bit-identical states; CELL evaluates the same collision
+ * (FP32: the same formulas one cell at a time, a different operation order).  A
+ * kind chosen by name runs as that kernel on every lattice; PAIR and CELL may take
+ * the wall rows into their one launch.  AUTO takes the fastest that gives the bits
+ * of the kind it stands for: where that is QUAD, lattices of at most 100,000 cells
+ * step in one launch of PAIR's kernel, and where it is PAIR, larger 16-bit lattices
+ * take four cells a thread.  Errors: LBM_EINVAL for an unknown kind or a grid the
+ * kind does not support. */
 int lbm_set_step_kernel(lbm_handle *h, int kind);
 
-/* The kernel later steps will run (AUTO resolved) into *kind.  Errors:
+/* The kind chosen into *kind; for AUTO the kind that it stands for, whose bits its
+ * steps give (a kind by name is also the kernel that runs).  Errors:
  * LBM_EINVAL for NULL pointers. */
 int lbm_get_step_kernel(const lbm_handle *h, int *kind);
 

@@ -627,11 +627,7 @@ bool staged_supported(const lbm_handle *h) {
     return h->nx % (16 / (int)h->elem) == 0 && tensor_map_encoder() != nullptr;
 }
 
-int resolve_kind(const lbm_handle *h) {
-    if (h->step_kind != LBM_KERNEL_AUTO) return h->step_kind;
-    if (h->elem == 2 && h->nx % 4 == 0) return LBM_KERNEL_QUAD;
-    return h->nx % 2 == 0 ? LBM_KERNEL_PAIR : LBM_KERNEL_CELL;
-}
+int resolve_kind(const lbm_handle *h) { return lbmk::resolve_kind(h->step_kind, (int)h->elem, h->nx); }
 
 // 4-d tensor map (x, y, z, q) of a lattice at `base`, box (BW, 2, 1, 1).
 template <class S>
@@ -715,16 +711,6 @@ void sponge_args(const lbm_handle *h, float &x0, float &inv, float &s3nu) {
     s3nu = L > 0 ? (float)(3.0 * h->sponge_nu) : 0.0f;
 }
 
-// Whether a step runs as one launch, wall blocks and interior blocks together,
-// or as an interior kernel with the wall rows on a side stream beside it.  Up to
-// about 100,000 cells all blocks of the one launch are resident at once and it
-// saves the fork and join (64x32x32: FP32 5.1 -> 4.4 us per step in a graph, FP16
-// 5.4 -> 4.8); beyond that the wall blocks, whose chain is the longer one, hold
-// up the interior ones that wait for their place (96x32x48: FP32 6.0 -> 6.5 us;
-// 400x40x32: 11.6 -> 12.6).
-constexpr long long kOneLaunchCells = 100000;
-bool one_launch(const lbm_handle *h) { return h->ncell <= kOneLaunchCells; }
-
 template <class S>
 cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
     using T = typename S::T;
@@ -762,30 +748,22 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
         tev1 = h->ev1[slot];
     }
     if (timed) cudaEventRecord(tev0, h->stream);
-    int kind = resolve_kind(h);
-    if (io.obj && kind != LBM_KERNEL_CELL) kind = LBM_KERNEL_PAIR;   // the kernel that sums the objective
-    // block (bx, BY), two cells a thread: 2 bx columns of two rows; bx = 32 where
-    // it covers the row with fewer empty columns (400 columns: 448 instead of 512,
-    // 11.4 -> 10.8 us per 400x40x32 FP32 step)
-    const int n32 = (h->nx + 63) / 64, wide = lbmk::STEP_THREADS / lbmk::BY;
-    const int bx = n32 % (wide / 32) ? 32 : wide;
-    const int nbx = (h->nx + 2 * bx - 1) / (2 * bx);
-    const dim3 block(bx, lbmk::BY);
-    const bool split = h->nx % 2 != 0 || kind == LBM_KERNEL_CELL;
-    const bool one = kind != LBM_KERNEL_STAGED && one_launch(h);
+    const lbmk::StepRoute r = lbmk::step_route(h->step_kind, io.obj != nullptr, (int)h->elem, h->nx, h->ny, h->nz);
+    const int rows = h->ny / lbmk::BY;                   // block rows
+    const dim3 block(r.bx, lbmk::BY);
     constexpr bool fp32 = std::is_same<S, lbmk::StoreF32>::value;
+    const bool cell32 = fp32 && r.kind == LBM_KERNEL_CELL;
     cudaError_t err = cudaSuccess;
-    const bool cell32 = fp32 && kind == LBM_KERNEL_CELL;
-    if (io.fw == h->d_fw) h->fw_side = !one;
-    if (cell32 && one) {
+    if (io.fw == h->d_fw) h->fw_side = !r.one;
+    if (cell32 && r.one) {
         if constexpr (fp32) {
-            const dim3 grid((h->nx + 31) / 32, h->ny / lbmk::BY, h->nz), cblock(32, lbmk::BY);
-            if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_ALL><<<grid, cblock, 0, h->stream>>>(a);
-            else lbmk::step_kernel<false, lbmk::CELLS_ALL><<<grid, cblock, 0, h->stream>>>(a);
+            const dim3 grid(r.nbx, rows, h->nz);
+            if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_ALL><<<grid, block, 0, h->stream>>>(a);
+            else lbmk::step_kernel<false, lbmk::CELLS_ALL><<<grid, block, 0, h->stream>>>(a);
         }
-    } else if (one) {
-        const dim3 grid(nbx, h->ny / lbmk::BY, h->nz);
-        if (!split) {
+    } else if (r.one) {
+        const dim3 grid(r.nbx, rows, h->nz);
+        if (!r.split) {
             if (io.stats) lbmk::step2_kernel<S, true, false, true><<<grid, block, 0, h->stream>>>(a);
             else lbmk::step2_kernel<S, false, false, true><<<grid, block, 0, h->stream>>>(a);
         } else if constexpr (!fp32) {
@@ -805,39 +783,34 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
         a.wall_planes = std::max(1, std::min(4, (int)(interior_us / 12.0)));
         const dim3 wgrid((h->nx + lbmk::WALL_THREADS - 1) / lbmk::WALL_THREADS,
                          (h->nz + a.wall_planes - 1) / a.wall_planes);
-        const int cx = h->nx >= 64 ? 64 : 32;
-        const dim3 cgrid((h->nx + cx - 1) / cx, h->ny / lbmk::BY, h->nz), cblock(cx, lbmk::BY);
         if (cell32) {
             if constexpr (fp32) {
-                const dim3 cw(cgrid.x, 2, cgrid.z);
-                if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_WALL><<<cw, cblock, 0, h->side>>>(a);
-                else lbmk::step_kernel<false, lbmk::CELLS_WALL><<<cw, cblock, 0, h->side>>>(a);
+                const dim3 cw(r.nbx, 2, h->nz);
+                if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_WALL><<<cw, block, 0, h->side>>>(a);
+                else lbmk::step_kernel<false, lbmk::CELLS_WALL><<<cw, block, 0, h->side>>>(a);
             }
         } else if (io.stats) lbmk::wall_kernel<S, true><<<wgrid, lbmk::WALL_THREADS, 0, h->side>>>(a);
         else lbmk::wall_kernel<S, false><<<wgrid, lbmk::WALL_THREADS, 0, h->side>>>(a);
         if ((err = cudaEventRecord(h->ev_join, h->side)) != cudaSuccess) return err;
-        const dim3 grid(nbx, (h->ny - 2) / lbmk::BY, h->nz);
+        const dim3 grid(r.nbx, rows - 1, h->nz);         // rows 1 .. ny-2
         if (cell32) {
             if constexpr (fp32) {
-                const dim3 ci(cgrid.x, cgrid.y - 2, cgrid.z);
+                const dim3 ci(r.nbx, rows - 2, h->nz);
                 if (ci.y == 0) { /* ny = 4: wall rows only */ }
-                else if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_INTERIOR><<<ci, cblock, 0, h->stream>>>(a);
-                else lbmk::step_kernel<false, lbmk::CELLS_INTERIOR><<<ci, cblock, 0, h->stream>>>(a);
+                else if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_INTERIOR><<<ci, block, 0, h->stream>>>(a);
+                else lbmk::step_kernel<false, lbmk::CELLS_INTERIOR><<<ci, block, 0, h->stream>>>(a);
             }
-        } else if (kind == LBM_KERNEL_STAGED) {
+        } else if (r.kind == LBM_KERNEL_STAGED) {
             err = io.stats ? launch_staged<S, true>(h, a, io.in) : launch_staged<S, false>(h, a, io.in);
-        } else if (kind == LBM_KERNEL_QUAD) {
-            const dim3 qgrid((h->nx + 127) / 128, (h->ny - 2) / lbmk::BY, h->nz), qblock(32, lbmk::BY);
-            if (io.stats) lbmk::step4_kernel<S, true, false><<<qgrid, qblock, 0, h->stream>>>(a);
-            else lbmk::step4_kernel<S, false, false><<<qgrid, qblock, 0, h->stream>>>(a);
-        } else if (!fp32 && !split && h->nx % 4 != 0) {
-            // 16-bit words are worth four cells a thread also where rows start on a pair
+        } else if (r.kind == LBM_KERNEL_QUAD && !r.even) {
+            if (io.stats) lbmk::step4_kernel<S, true, false><<<grid, block, 0, h->stream>>>(a);
+            else lbmk::step4_kernel<S, false, false><<<grid, block, 0, h->stream>>>(a);
+        } else if (r.kind == LBM_KERNEL_QUAD) {
             if constexpr (!fp32) {
-                const dim3 qgrid((h->nx + 127) / 128, (h->ny - 2) / lbmk::BY, h->nz), qblock(32, lbmk::BY);
-                if (io.stats) lbmk::step4_kernel<S, true, true><<<qgrid, qblock, 0, h->stream>>>(a);
-                else lbmk::step4_kernel<S, false, true><<<qgrid, qblock, 0, h->stream>>>(a);
+                if (io.stats) lbmk::step4_kernel<S, true, true><<<grid, block, 0, h->stream>>>(a);
+                else lbmk::step4_kernel<S, false, true><<<grid, block, 0, h->stream>>>(a);
             }
-        } else if (!split) {
+        } else if (!r.split) {
             if (io.stats) lbmk::step2_kernel<S, true, false, false><<<grid, block, 0, h->stream>>>(a);
             else lbmk::step2_kernel<S, false, false, false><<<grid, block, 0, h->stream>>>(a);
         } else if constexpr (!fp32) {

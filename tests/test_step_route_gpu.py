@@ -1,0 +1,60 @@
+"""What a step launches, counted by the library itself, and lattices on which the
+kernels of named and automatic choice differ, against each other."""
+import ctypes as ct
+
+import numpy as np
+import pytest
+
+from gpu_helpers import make_pair, set_both
+from paper_2304_04214_gb300.inputs import noise
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _launches(g, steps):
+    """Kernels the handle launches in so many steps (a read starts the count again)."""
+    ms, nk, n = ct.c_double(), ct.c_long(), ct.c_long()
+    g.lib.lbm_profile_read(g.h, ct.byref(ms), ct.byref(nk), ct.byref(n))
+    g.step(steps)
+    g.lib.lbm_profile_read(g.h, ct.byref(ms), ct.byref(nk), ct.byref(n))
+    return n.value
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16", "bf16", "fp16row"])
+def test_quad_by_name_runs_beside_the_wall_kernel_on_any_lattice(precision):
+    """Small lattices too: QUAD has no wall rows, so a step by that name is two
+    launches, where PAIR and AUTO take one."""
+    from paper_2304_04214_gb300.channel import LBMChannel
+    g = LBMChannel(64, 16, 8, n_modes=0, inlet=False, precision=precision)
+    for kernel, want in (("quad", 2), ("pair", 1), ("auto", 1), ("staged", 2), ("cell", 1)):
+        g.step_kernel = kernel
+        assert _launches(g, 4) == 4 * want, kernel
+    g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp16", "bf16", "fp16row"])
+@pytest.mark.parametrize("shape", [(126, 30, 28), (66, 40, 42), (602, 8, 22)])
+def test_pair_by_name_gives_the_bits_of_four_cells_a_thread(shape, precision):
+    """16-bit lattices of nx = 4m + 2 above 100,000 cells: AUTO takes four cells a
+    thread, PAIR two; the last thread of a row at a warp's end, in its middle and
+    between."""
+    nx, ny, nz = shape
+    assert nx * ny * nz > 100000
+    got = []
+    for kernel in ("auto", "pair"):
+        o, g = make_pair(nx, ny, nz, n_modes=8, seed=6, precision=precision, stats=1)
+        g.step_kernel = kernel
+        set_both(o, g, o.state() * (1.0 + 0.02 * noise((19, nz, ny, nx), seed=8)))
+        g.set_sponge(nx // 10, 0.05)
+        g.step(3)
+        got.append((g.populations(), g.utau(), g.stats()[0]))
+        g.close()
+    for x, y in zip(*got):
+        assert np.array_equal(x, y)
