@@ -144,8 +144,8 @@ int lbm_bind_memory(lbm_handle *h, void *dev_ptr, size_t bytes);
  * regularized inlet (steps 6-8) and the collision (step 15); the wall-row
  * kernel (rows 0 and ny-1, on a side stream forked from and joined back into
  * the handle's stream) does the same for the first off-wall cells with the
- * wall model (steps 9-14).  (Lattices of at most 100,000 cells: one kernel for
- * all rows, the same arithmetic.)
+ * wall model (steps 9-14).  (Lattices of at most 100,000 cells, if the device
+ * holds all their blocks at once: one kernel for all rows, the same arithmetic.)
  * With CUDA graphs on (the default, lbm_set_graphs), whole periods of the STG
  * ring (64 steps where the inlet plane allows) that fit in n are launched as
  * one graph each, built the first time a period's launch state occurs; the
@@ -219,9 +219,9 @@ int lbm_set_stream(lbm_handle *h, void *cuda_stream);
  * (FP32: the same formulas one cell at a time, a different operation order).  A
  * kind chosen by name runs as that kernel on every lattice; PAIR and CELL may take
  * the wall rows into their one launch.  AUTO takes the fastest that gives the bits
- * of the kind it stands for: where that is QUAD, lattices of at most 100,000 cells
- * step in one launch of PAIR's kernel, and where it is PAIR, larger 16-bit lattices
- * take four cells a thread.  Errors: LBM_EINVAL for an unknown kind or a grid the
+ * of the kind it stands for: where that is QUAD, lattices that step in one launch
+ * (lbm_step) take PAIR's kernel, and where it is PAIR, larger 16-bit lattices take
+ * four cells a thread.  Errors: LBM_EINVAL for an unknown kind or a grid the
  * kind does not support. */
 int lbm_set_step_kernel(lbm_handle *h, int kind);
 

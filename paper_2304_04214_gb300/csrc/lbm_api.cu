@@ -177,6 +177,7 @@ struct lbm_handle {
     std::vector<double> prof_U, prof_R;
     double *d_tw = nullptr;                // [2][nx] wall-shear scratch
     long long *d_gt0 = nullptr;            // start time of the refill inside a graph
+    int sms = 0;                           // of the bound memory's device
     bool fw_side = false;                  // d_fw was last written by the side-stream wall kernel
     cudaEvent_t ev_shear = nullptr;        // wall-shear reduction done on the side stream
     // the wall-row kernel runs beside the interior kernel on a side stream,
@@ -627,7 +628,7 @@ bool staged_supported(const lbm_handle *h) {
     return h->nx % (16 / (int)h->elem) == 0 && tensor_map_encoder() != nullptr;
 }
 
-int resolve_kind(const lbm_handle *h) { return lbmk::resolve_kind(h->step_kind, (int)h->elem, h->nx); }
+int resolve_kind(const lbm_handle *h) { return lbmk::resolve_kind(h->step_kind, h->opts.precision, h->nx); }
 
 // 4-d tensor map (x, y, z, q) of a lattice at `base`, box (BW, 2, 1, 1).
 template <class S>
@@ -748,7 +749,8 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
         tev1 = h->ev1[slot];
     }
     if (timed) cudaEventRecord(tev0, h->stream);
-    const lbmk::StepRoute r = lbmk::step_route(h->step_kind, io.obj != nullptr, (int)h->elem, h->nx, h->ny, h->nz);
+    const lbmk::StepRoute r = lbmk::step_route(h->step_kind, io.obj != nullptr, h->opts.precision, h->nx, h->ny,
+                                                 h->nz, h->sms);
     const int rows = h->ny / lbmk::BY;                   // block rows
     const dim3 block(r.bx, lbmk::BY);
     constexpr bool fp32 = std::is_same<S, lbmk::StoreF32>::value;
@@ -1306,6 +1308,7 @@ int lbm_bind_memory(lbm_handle *h, void *dev_ptr, size_t bytes) {
         return cuda_fail(cudaGetLastError());
     }
     h->pin_shear = (double *)((char *)h->pin_stage + stage_bytes);
+    h->sms = device_sms();
     Arena ar;
     ar.base = (char *)h->mem;
     ar.guard = h->guard_bytes;

@@ -22,54 +22,68 @@ struct StepRoute {
     int bx, nbx;   // threads of a block along x, blocks along x
 };
 
+// Bytes of a stored population.
+inline int elem_bytes(int precision) { return precision == LBM_FP32 ? 4 : 2; }
+
 // The variant that `kind` stands for: AUTO is QUAD for the 16-bit storages where
 // nx is a multiple of four, else PAIR (nx even), else CELL.
-inline int resolve_kind(int kind, int elem, int nx) {
+inline int resolve_kind(int kind, int precision, int nx) {
     if (kind != LBM_KERNEL_AUTO) return kind;
-    if (elem == 2 && nx % 4 == 0) return LBM_KERNEL_QUAD;
+    if (elem_bytes(precision) == 2 && nx % 4 == 0) return LBM_KERNEL_QUAD;
     return nx % 2 == 0 ? LBM_KERNEL_PAIR : LBM_KERNEL_CELL;
 }
 
-// Up to about 100,000 cells all blocks of the one launch are resident at once and
-// it saves the fork and join (64x32x32: FP32 5.1 -> 4.4 us per step in a graph, FP16
-// 5.4 -> 4.8); beyond that the wall blocks, whose chain is the longer one, hold
-// up the interior ones that wait for their place (96x32x48: FP32 6.0 -> 6.5 us;
-// 400x40x32: 11.6 -> 12.6).
+// A step in one launch saves the fork and join of the side stream (64x32x32 in a
+// graph: FP32 4.9 -> 4.4 us, FP16 5.1 -> 4.6) as long as all its blocks are resident
+// at once: the wall blocks, whose chain is the longer one, come first, and blocks
+// that wait for their place hold up the step (us, one launch / two: 66x32x47 FP16
+// 6.8 / 5.9, 8x110x110 FP32 16.9 / 15.7, 33x40x70 FP32 7.7 / 6.4; all resident: 48x48x42
+// 5.66 / 5.70, 130x24x32 5.8 / 6.1).  The kernels' launch bounds keep this many
+// threads resident on an SM; larger lattices fill the chip without it.
 constexpr long long ONE_LAUNCH_CELLS = 100000;
+constexpr int ONE_BLOCKS_PER_SM = 4;
 
 // kind: the variant chosen (LBM_KERNEL_AUTO or a name); objective: the step sums
-// an adjoint window's objective, which the CELL and PAIR kernels can; elem: bytes of
-// a stored population.  A variant chosen by name runs as that kernel on every
-// lattice it accepts.  AUTO takes what is fastest and gives the same bits: PAIR's
-// kernel for a step in one launch, QUAD's for larger 16-bit lattices of even nx.
-inline StepRoute step_route(int kind, bool objective, int elem, int nx, int ny, int nz) {
+// an adjoint window's objective, which the CELL and PAIR kernels can; precision: the
+// storage; sms: SMs of the device.  A variant chosen by name runs as that kernel on
+// every lattice it accepts.  AUTO takes what is fastest and gives the same bits:
+// PAIR's kernel for a step in one launch, QUAD's for larger 16-bit lattices of even
+// nx.
+inline StepRoute step_route(int kind, bool objective, int precision, int nx, int ny, int nz, int sms) {
     StepRoute r;
+    const int elem = elem_bytes(precision);
     const bool named_quad = kind == LBM_KERNEL_QUAD && !objective;
-    r.kind = resolve_kind(kind, elem, nx);
+    r.kind = resolve_kind(kind, precision, nx);
     if (objective && r.kind != LBM_KERNEL_CELL) r.kind = LBM_KERNEL_PAIR;
     r.split = r.kind == LBM_KERNEL_CELL && elem == 2;
-    r.one = (long long)nx * ny * nz <= ONE_LAUNCH_CELLS && r.kind != LBM_KERNEL_STAGED && !named_quad;
-    if (r.one && r.kind == LBM_KERNEL_QUAD) r.kind = LBM_KERNEL_PAIR;
     r.even = false;
-    if (!r.one && kind == LBM_KERNEL_AUTO && r.kind == LBM_KERNEL_PAIR && elem == 2) {
+    const bool cell32 = r.kind == LBM_KERNEL_CELL && elem == 4;
+    auto blocks = [&](int bx, int cells) { r.bx = bx; r.nbx = (nx + bx * cells - 1) / (bx * cells); };
+    // two cells a thread: 2 bx columns of two rows; bx = 32 where it covers the row
+    // with fewer empty columns (400 columns: 448 instead of 512, 11.4 -> 10.8 us per
+    // 400x40x32 FP32 step)
+    const int n32 = (nx + 63) / 64, wide = STEP_THREADS / BY, pair_bx = n32 % (wide / 32) ? 32 : wide;
+    auto resident = [&] {
+        return (long long)r.nbx * r.bx * ny * nz <= (long long)sms * ONE_BLOCKS_PER_SM * STEP_THREADS;
+    };
+    if (cell32) blocks(32, 1);
+    else blocks(pair_bx, 2);
+    // without interior rows there is nothing for wall rows to run beside (999x4x24 FP32
+    // 5.7 / 6.9), and QUAD's warps of 128 columns are mostly empty on rows of up to 64
+    // (16x60x100 FP16 10.0 / 11.4, 36x50x55 7.0 / 7.0, BF16 7.2 / 7.6)
+    r.one = (long long)nx * ny * nz <= ONE_LAUNCH_CELLS && r.kind != LBM_KERNEL_STAGED && !named_quad &&
+            (resident() || ny == 2 * BY || (r.kind == LBM_KERNEL_QUAD && nx <= 64));
+    if (r.one) {
+        if (r.kind == LBM_KERNEL_QUAD) r.kind = LBM_KERNEL_PAIR;
+        return r;
+    }
+    if (cell32) blocks(nx < 64 ? 32 : 64, 1);
+    if (kind == LBM_KERNEL_AUTO && r.kind == LBM_KERNEL_PAIR && elem == 2) {
         // 16-bit words are worth four cells a thread also where rows start on a pair
         r.kind = LBM_KERNEL_QUAD;
         r.even = true;
     }
-    if (r.kind == LBM_KERNEL_CELL && elem == 4) {
-        r.bx = r.one || nx < 64 ? 32 : 64;
-        r.nbx = (nx + r.bx - 1) / r.bx;
-    } else if (r.kind == LBM_KERNEL_QUAD) {
-        r.bx = 32;
-        r.nbx = (nx + 4 * r.bx - 1) / (4 * r.bx);
-    } else {
-        // two cells a thread: 2 bx columns of two rows; bx = 32 where it covers
-        // the row with fewer empty columns (400 columns: 448 instead of 512, 11.4 ->
-        // 10.8 us per 400x40x32 FP32 step)
-        const int n32 = (nx + 63) / 64, wide = STEP_THREADS / BY;
-        r.bx = n32 % (wide / 32) ? 32 : wide;
-        r.nbx = (nx + 2 * r.bx - 1) / (2 * r.bx);
-    }
+    if (r.kind == LBM_KERNEL_QUAD) blocks(32, 4);
     return r;
 }
 

@@ -24,16 +24,19 @@ def route(tmp_path_factory):
     if not cxx:
         pytest.skip("no C++ compiler")
     d = tmp_path_factory.mktemp("route")
-    (d / "r.cpp").write_text('#include "lbm_route.h"\nextern "C" void route(int kind, int obj, int elem, int nx, int ny, '
-                             'int nz, lbmk::StepRoute *r) { *r = lbmk::step_route(kind, obj, elem, nx, ny, nz); }\n')
+    (d / "r.cpp").write_text('#include "lbm_route.h"\nextern "C" void route(int kind, int obj, int precision, int nx, '
+                             'int ny, int nz, int sms, lbmk::StepRoute *r) '
+                             '{ *r = lbmk::step_route(kind, obj, precision, nx, ny, nz, sms); }\n')
     so = str(d / "r.so")
     subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", "-I", build.CSRC, "-I", build.INCLUDE,
                     str(d / "r.cpp"), "-o", so], check=True)
     lib = ct.CDLL(so)
 
-    def f(kind, elem, shape, obj=False):
+    def f(kind, elem, shape, obj=False, precision=None, sms=152):
         r = Route()
-        lib.route(kind, int(obj), elem, *shape, ct.byref(r))
+        if precision is None:
+            precision = _abi.LBM_FP32 if elem == 4 else _abi.LBM_FP16_DEV
+        lib.route(kind, int(obj), precision, *shape, sms, ct.byref(r))
         return r
     return f
 
@@ -68,3 +71,27 @@ def test_blocks_cover_the_row_once(route, shape, elem):
             assert not obj or r.kind in (CELL, PAIR)
             assert nx % 2 == 0 or r.kind == CELL
             assert r.kind != QUAD or nx % 4 == 0 or (r.even and elem == 2)
+
+
+@pytest.mark.parametrize("elem,shape,one", [
+    (4, (64, 32, 32), True), (2, (64, 32, 32), True), (2, (48, 48, 42), True), (4, (130, 24, 32), True),
+    (2, (128, 32, 24), True), (4, (63, 32, 32), True),
+    # more blocks than the device holds at once
+    (2, (66, 32, 47), False), (4, (8, 110, 110), False), (4, (20, 50, 98), False), (2, (34, 48, 60), False),
+    (2, (72, 40, 34), False), (4, (33, 40, 70), False), (4, (97, 32, 32), False), (2, (65, 32, 47), False),
+    # wall rows only; QUAD's lattices of narrow rows; above the cell count
+    (4, (999, 4, 24), True), (2, (16, 60, 100), True), (4, (128, 32, 32), False), (2, (96, 32, 48), False)])
+def test_one_launch_where_its_blocks_are_resident(route, elem, shape, one):
+    assert bool(route(AUTO, elem, shape).one) == one
+
+
+def test_one_launch_follows_the_size_of_the_device(route):
+    """The same lattice on fewer SMs; and never more blocks than fit, but for wall
+    rows alone and QUAD's narrow lattices."""
+    assert route(AUTO, 4, (64, 32, 32), sms=64).one and not route(AUTO, 4, (64, 32, 32), sms=63).one
+    for nx in range(2, 200):
+        for ny, nz in ((6, 60), (16, 40), (40, 40), (90, 90)):
+            for elem in (2, 4):
+                r = route(AUTO, elem, (nx, ny, nz))
+                if r.one and not (elem == 2 and nx % 4 == 0 and nx <= 64):
+                    assert r.bx * r.nbx * ny * nz <= 152 * 512

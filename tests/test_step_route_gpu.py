@@ -58,3 +58,38 @@ def test_pair_by_name_gives_the_bits_of_four_cells_a_thread(shape, precision):
         g.close()
     for x, y in zip(*got):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("precision,shape,want", [
+    ("fp16", (66, 32, 47), 2), ("fp32", (8, 110, 110), 2), ("fp32", (33, 40, 70), 2), ("bf16", (34, 48, 60), 2),
+    ("fp32", (48, 48, 42), 1), ("fp16row", (64, 32, 32), 1), ("fp16", (129, 16, 40), 1)])
+def test_lattices_whose_blocks_do_not_fit_at_once_step_in_two_launches(precision, shape, want):
+    from paper_2304_04214_gb300.channel import LBMChannel
+    g = LBMChannel(*shape, n_modes=0, inlet=False, precision=precision)
+    assert _launches(g, 4) == 4 * want
+    g.close()
+
+
+@pytest.mark.parametrize("inlet", [True, False])
+@pytest.mark.parametrize("precision", ["fp32", "fp16", "bf16", "fp16row"])
+@pytest.mark.parametrize("nx,ny,nz", [(65, 16, 8), (129, 6, 11), (64, 16, 8), (66, 8, 15), (33, 12, 9), (301, 4, 7)])
+def test_one_launch_and_two_give_the_same_bits(nx, ny, nz, precision, inlet):
+    """A state that repeats in z with a period of nz planes (an inlet without modes is
+    uniform in z) stays so, plane for plane, in a lattice of many periods: the short
+    one steps in one launch, the long one with its wall rows on the side stream.
+    Three steps (both traversal directions), with statistics."""
+    from paper_2304_04214_gb300.channel import LBMChannel
+    reps = 100000 // (nx * ny * nz) + 1
+    f = None
+    got = []
+    for n in (1, reps):
+        g = LBMChannel(nx, ny, n * nz, n_modes=0, inlet=inlet, precision=precision, stats_every=1)
+        if f is None:
+            f = g.populations() * (1.0 + 0.02 * noise((19, nz, ny, nx), seed=8))
+        g.set_populations(np.tile(f, (1, n, 1, 1)))
+        g.step(3)
+        got.append((g.populations(), g.utau()))
+        g.close()
+    (f1, u1), (f2, u2) = got
+    assert np.array_equal(np.tile(f1, (1, reps, 1, 1)), f2)
+    assert np.array_equal(np.tile(u1, (1, reps, 1)), u2)
