@@ -220,9 +220,9 @@ int lbm_set_stream(lbm_handle *h, void *cuda_stream);
  * kind chosen by name runs as that kernel on every lattice; PAIR and CELL may take
  * the wall rows into their one launch.  AUTO takes the fastest that gives the bits
  * of the kind it stands for: where that is QUAD, lattices that step in one launch
- * (lbm_step) take PAIR's kernel, and where it is PAIR, larger 16-bit lattices take
- * four cells a thread.  Errors: LBM_EINVAL for an unknown kind or a grid the
- * kind does not support. */
+ * (lbm_step) take PAIR's kernel, and where it is PAIR, some larger lattices of nx =
+ * 4m + 2 in the row-base storages take four cells a thread.  Errors: LBM_EINVAL for
+ * an unknown kind or a grid the kind does not support. */
 int lbm_set_step_kernel(lbm_handle *h, int kind);
 
 /* The kind chosen into *kind; for AUTO the kind that it stands for, whose bits its

@@ -808,7 +808,7 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
             if (io.stats) lbmk::step4_kernel<S, true, false><<<grid, block, 0, h->stream>>>(a);
             else lbmk::step4_kernel<S, false, false><<<grid, block, 0, h->stream>>>(a);
         } else if (r.kind == LBM_KERNEL_QUAD) {
-            if constexpr (!fp32) {
+            if constexpr (S::ROWBASE) {
                 if (io.stats) lbmk::step4_kernel<S, true, true><<<grid, block, 0, h->stream>>>(a);
                 else lbmk::step4_kernel<S, false, true><<<grid, block, 0, h->stream>>>(a);
             }

@@ -47,8 +47,8 @@ constexpr int ONE_BLOCKS_PER_SM = 4;
 // an adjoint window's objective, which the CELL and PAIR kernels can; precision: the
 // storage; sms: SMs of the device.  A variant chosen by name runs as that kernel on
 // every lattice it accepts.  AUTO takes what is fastest and gives the same bits:
-// PAIR's kernel for a step in one launch, QUAD's for larger 16-bit lattices of even
-// nx.
+// PAIR's kernel for a step in one launch, QUAD's also on some larger lattices of
+// nx = 4m + 2.
 inline StepRoute step_route(int kind, bool objective, int precision, int nx, int ny, int nz, int sms) {
     StepRoute r;
     const int elem = elem_bytes(precision);
@@ -78,8 +78,13 @@ inline StepRoute step_route(int kind, bool objective, int precision, int nx, int
         return r;
     }
     if (cell32) blocks(nx < 64 ? 32 : 64, 1);
-    if (kind == LBM_KERNEL_AUTO && r.kind == LBM_KERNEL_PAIR && elem == 2) {
-        // 16-bit words are worth four cells a thread also where rows start on a pair
+    const bool rowbase = precision == LBM_BF16_DEV || precision == LBM_FP16_ROW;
+    if (kind == LBM_KERNEL_AUTO && r.kind == LBM_KERNEL_PAIR && rowbase && n32 % 2 == 0) {
+        // Four cells a thread also where rows start on a pair of them, for the
+        // storages whose row bases a thread then loads half as often, and if the warps
+        // of 128 columns leave no more of them empty than two cells a thread do (us,
+        // four / two cells: 602x60x48 BF16 28.0 / 28.7, 66x60x60 9.3 / 9.7, 222x60x60 FP16 row
+        // 15.1 / 15.5; FP16 602x60x48 27.2 / 26.6; 34x60x60 BF16 9.2 / 7.3, 386x96x96 64.4 / 61.8)
         r.kind = LBM_KERNEL_QUAD;
         r.even = true;
     }

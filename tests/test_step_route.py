@@ -95,3 +95,18 @@ def test_one_launch_follows_the_size_of_the_device(route):
                 r = route(AUTO, elem, (nx, ny, nz))
                 if r.one and not (elem == 2 and nx % 4 == 0 and nx <= 64):
                     assert r.bx * r.nbx * ny * nz <= 152 * 512
+
+
+FP16, BF16, ROW = _abi.LBM_FP16_DEV, _abi.LBM_BF16_DEV, _abi.LBM_FP16_ROW
+
+
+@pytest.mark.parametrize("shape,precision,even", [
+    ((602, 60, 48), BF16, True), ((602, 60, 48), ROW, True), ((66, 60, 60), BF16, True), ((126, 30, 28), ROW, True),
+    ((222, 60, 60), ROW, True),
+    # plain FP16, and rows that warps of 128 columns leave emptier than blocks of 64 or 128
+    ((602, 60, 48), FP16, False), ((34, 60, 60), BF16, False), ((18, 100, 100), ROW, False),
+    ((130, 48, 48), BF16, False), ((386, 96, 96), ROW, False), ((1026, 8, 14), BF16, False)])
+def test_four_cells_a_thread_on_rows_of_pairs(route, shape, precision, even):
+    r = route(AUTO, 2, shape, precision=precision)
+    assert bool(r.even) == even and r.kind == (QUAD if even else PAIR) and not r.one
+    assert not even or r.nbx * 128 <= -(-shape[0] // 64) * 64
