@@ -68,6 +68,10 @@ inline StepRoute step_route(int kind, bool objective, int precision, int nx, int
     };
     if (cell32) blocks(32, 1);
     else blocks(pair_bx, 2);
+    // narrow odd rows: 32 columns to a block instead of 64 (21x100x100 FP16 15.2 -> 9.9 us;
+    // one cell a thread 13.2), unless the wider blocks are all resident as it is
+    // (21x16x30: 4.4 with 64, 4.9 with 32)
+    if (r.split && nx <= 32 && !resident()) blocks(16, 2);
     // without interior rows there is nothing for wall rows to run beside (999x4x24 FP32
     // 5.7 / 6.9), and QUAD's warps of 128 columns are mostly empty on rows of up to 64
     // (16x60x100 FP16 10.0 / 11.4, 36x50x55 7.0 / 7.0, BF16 7.2 / 7.6)

@@ -110,3 +110,12 @@ def test_four_cells_a_thread_on_rows_of_pairs(route, shape, precision, even):
     r = route(AUTO, 2, shape, precision=precision)
     assert bool(r.even) == even and r.kind == (QUAD if even else PAIR) and not r.one
     assert not even or r.nbx * 128 <= -(-shape[0] // 64) * 64
+
+
+@pytest.mark.parametrize("shape,bx,one", [
+    ((21, 16, 30), 32, True), ((31, 40, 40), 32, True),      # resident in blocks of 64 columns
+    ((21, 48, 90), 16, True), ((29, 58, 58), 16, True),
+    ((21, 100, 100), 16, False), ((33, 100, 100), 32, False), ((27, 4, 1000), 16, False)])
+def test_narrow_odd_rows_of_16_bit_lattices(route, shape, bx, one):
+    r = route(AUTO, 2, shape)
+    assert r.split and r.bx == bx and bool(r.one) == one

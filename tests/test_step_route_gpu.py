@@ -93,3 +93,25 @@ def test_one_launch_and_two_give_the_same_bits(nx, ny, nz, precision, inlet):
     (f1, u1), (f2, u2) = got
     assert np.array_equal(np.tile(f1, (1, reps, 1, 1)), f2)
     assert np.array_equal(np.tile(u1, (1, reps, 1)), u2)
+
+
+@pytest.mark.parametrize("precision", ["fp16", "bf16", "fp16row"])
+@pytest.mark.parametrize("nx,ny,nz", [(3, 6, 9), (15, 4, 5), (21, 8, 11), (31, 16, 10)])
+def test_narrow_odd_rows_give_the_same_bits_in_blocks_of_any_width(nx, ny, nz, precision):
+    """As above for rows of at most 32 cells: the short lattice in blocks of 64 columns,
+    the middle one in one launch of blocks of 32, the long one in two launches."""
+    test_one_launch_and_two_give_the_same_bits(nx, ny, nz, precision, True)
+    from paper_2304_04214_gb300.channel import LBMChannel
+    f = None
+    got = []
+    for n in (1, 100000 // (32 * ny * nz)):
+        g = LBMChannel(nx, ny, n * nz, n_modes=0, precision=precision)
+        if f is None:
+            f = g.populations() * (1.0 + 0.02 * noise((19, nz, ny, nx), seed=8))
+        g.set_populations(np.tile(f, (1, n, 1, 1)))
+        g.step(3)
+        got.append((g.populations(), g.utau()))
+        g.close()
+    n = got[1][0].shape[1] // nz
+    assert np.array_equal(np.tile(got[0][0], (1, n, 1, 1)), got[1][0])
+    assert np.array_equal(np.tile(got[0][1], (1, n, 1)), got[1][1])
