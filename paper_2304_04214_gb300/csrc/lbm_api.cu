@@ -793,8 +793,13 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
                 if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_WALL><<<cw, block, 0, h->side>>>(a);
                 else lbmk::step_kernel<false, lbmk::CELLS_WALL><<<cw, block, 0, h->side>>>(a);
             }
-        } else if (io.stats) lbmk::wall_kernel<S, true><<<wgrid, wbx, 0, h->side>>>(a);
-        else lbmk::wall_kernel<S, false><<<wgrid, wbx, 0, h->side>>>(a);
+        } else if (r.split) {
+            if constexpr (!fp32) {
+                if (io.stats) lbmk::wall_kernel<S, true, true><<<wgrid, wbx, 0, h->side>>>(a);
+                else lbmk::wall_kernel<S, false, true><<<wgrid, wbx, 0, h->side>>>(a);
+            }
+        } else if (io.stats) lbmk::wall_kernel<S, true, false><<<wgrid, wbx, 0, h->side>>>(a);
+        else lbmk::wall_kernel<S, false, false><<<wgrid, wbx, 0, h->side>>>(a);
         if ((err = cudaEventRecord(h->ev_join, h->side)) != cudaSuccess) return err;
         const dim3 grid(r.nbx, rows - 1, h->nz);         // rows 1 .. ny-2
         if (cell32) {
