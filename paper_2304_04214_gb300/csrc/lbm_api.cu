@@ -805,7 +805,7 @@ cudaError_t launch_step_t(lbm_handle *h, const StepIO &io) {
         if (cell32) {
             if constexpr (fp32) {
                 const dim3 ci(r.nbx, rows - 2, h->nz);
-                if (ci.y == 0) { /* ny = 4: wall rows only */ }
+                if (ci.y == 0) h->launches -= 1;         // ny = 4: wall rows only
                 else if (io.stats) lbmk::step_kernel<true, lbmk::CELLS_INTERIOR><<<ci, block, 0, h->stream>>>(a);
                 else lbmk::step_kernel<false, lbmk::CELLS_INTERIOR><<<ci, block, 0, h->stream>>>(a);
             }

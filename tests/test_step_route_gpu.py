@@ -115,3 +115,11 @@ def test_narrow_odd_rows_give_the_same_bits_in_blocks_of_any_width(nx, ny, nz, p
     n = got[1][0].shape[1] // nz
     assert np.array_equal(np.tile(got[0][0], (1, n, 1, 1)), got[1][0])
     assert np.array_equal(np.tile(got[0][1], (1, n, 1)), got[1][1])
+
+
+def test_wall_rows_alone_are_one_launch():
+    """Odd FP32 lattices of ny = 4 above 100,000 cells: no interior kernel, none counted."""
+    from paper_2304_04214_gb300.channel import LBMChannel
+    g = LBMChannel(1001, 4, 30, n_modes=0, inlet=False)
+    assert _launches(g, 4) == 4
+    g.close()
