@@ -21,7 +21,7 @@ def lib(tmp_path_factory):
         pytest.skip("no C++ compiler")
     d = tmp_path_factory.mktemp("newton")
     (d / "n.cpp").write_text('#include "lbm_newton.h"\nextern "C" {\n'
-                             'double e(double x) { return lbmk::exp_neg_d(x); }\n'
+                             'double e(double x) { double p; return lbmk::exp_neg_d(x, p); }\n'
                              'double l(double z) { return lbmk::log1p_d(z); }\n'
                              'float s(float uhat, float y1, float kap, float B, float guess, int *ok) '
                              '{ bool o; const float u = lbmk::solve_utau_d(uhat, y1, kap, B, guess, &o); *ok = o; '
