@@ -34,7 +34,7 @@ inline int resolve_kind(int kind, int precision, int nx) {
 }
 
 // A step in one launch saves the fork and join of the side stream (64x32x32 in a
-// graph: FP32 4.9 -> 4.4 us, FP16 5.1 -> 4.6) as long as all its blocks are resident
+// graph: FP32 5.4 -> 4.5 us, FP16 5.5 -> 4.7) as long as all its blocks are resident
 // at once: the wall blocks, whose chain is the longer one, come first, and blocks
 // that wait for their place hold up the step (us, one launch / two: 66x32x47 FP16
 // 6.8 / 5.9, 8x110x110 FP32 16.9 / 15.7, 33x40x70 FP32 7.7 / 6.4; all resident: 48x48x42
