@@ -106,7 +106,8 @@ class LBMChannel:
 
     @property
     def step_kernel(self):
-        """The step kernel later steps run: 'cell', 'pair', 'quad' or 'staged'."""
+        """The step kernel later steps run: 'cell', 'pair', 'quad' or 'staged'; chosen
+        automatically, the one whose bits they give (lbm_set_step_kernel)."""
         k = ct.c_int()
         _abi.check(self.lib.lbm_get_step_kernel(self.h, ct.byref(k)), "lbm_get_step_kernel")
         return {v: n for n, v in _abi.KERNELS.items()}[k.value]
